@@ -4,7 +4,7 @@
 // plain BF16 writer for the comparison cache.
 //
 // A block of nine warps writes a few tokens: warp g quantises group g (64
-// coordinates) of four tokens at a time, eight lanes per token with eight
+// coordinates) of four or sixteen tokens, eight lanes per token with eight
 // coordinates (16 bytes) each. A warp then reads four whole 128-byte lines and,
 // where the tokens take consecutive slots (a prefill), writes their code rows
 // and scales as contiguous runs; the bit width and the scale format are uniform
@@ -90,68 +90,66 @@ __device__ __forceinline__ void codes8(const uint32_t (&w)[4], float s, float y,
   }
 }
 
-// Looks up and validates the destination of token i. Returns null (after
+// Looks up and validates the destination of token i: its block id, or -1 (after
 // recording the error) when the token cannot be written.
-__device__ __forceinline__ uint8_t* token_block(uint8_t* pool, size_t block_bytes, int num_blocks,
-                                                const int32_t* seq_ids, const int32_t* positions,
-                                                int i, const int32_t* table, int num_seqs,
-                                                int max_blocks, uint32_t* dev_err, int& slot) {
-  const int seq = seq_ids != nullptr ? seq_ids[i] : i;
-  const int pos = positions[i];
+__device__ __forceinline__ int token_block(int num_blocks, const int32_t* seq_ids, const int32_t* positions, int i,
+                                           const int32_t* table, int num_seqs, int max_blocks, uint32_t* dev_err,
+                                           int& seq, int& pos) {
+  seq = seq_ids != nullptr ? seq_ids[i] : i;
+  pos = positions[i];
   if (seq < 0 || seq >= num_seqs) {
     report(dev_err, QMLA_DEVERR_BAD_SEQ);
-    return nullptr;
+    return -1;
   }
   if (pos < 0 || pos >= max_blocks * kBlockTokens) {
     report(dev_err, QMLA_DEVERR_BAD_POSITION);
-    return nullptr;
+    return -1;
   }
   const int blk = table[static_cast<size_t>(seq) * max_blocks + pos / kBlockTokens];
   if (blk < 0 || blk >= num_blocks) {
     report(dev_err, QMLA_DEVERR_BAD_BLOCK);
-    return nullptr;
+    return -1;
   }
-  slot = pos % kBlockTokens;
-  return pool + static_cast<size_t>(blk) * block_bytes;
+  return blk;
 }
 
 // Sink/recent BF16 protection rows (App. C.5, "BF16 protection and cache
 // lifecycle"): position p of a request whose length after this write is L goes
-// to row p when p < 4 and to row 4 + p mod 128 when p >= L - 128. Each lane
-// stores its own 16 bytes, piece `piece` (0..71) of the token's 1152.
-__device__ __forceinline__ void protect_piece(uint4* prot, const uint4& v, int piece, int seq, int pos, int L) {
-  uint4* base = prot + static_cast<size_t>(seq) * kProtRows * (kDqk * 2 / 16) + piece;
-  if (pos < kSinkTokens) base[pos * (kDqk * 2 / 16)] = v;
-  if (pos >= L - kRecentTokens) base[(kSinkTokens + pos % kRecentTokens) * (kDqk * 2 / 16)] = v;
-}
+// to row p when p < 4 and to row 4 + p mod 128 when p >= L - 128; each lane stores
+// its own 16 bytes of the token's 1152.
 
 constexpr int kAppendThreads = kGroups * 32;
 
 // Quantises and packs n tokens. CB: content bits (4, 2) or kC4R4 for the paper's
-// page (INT4 codes). NT: tokens per lane (a block writes 4 NT). VEC: latent and
-// k_pe are 16-byte aligned (one 16-byte load per lane, else four 4-byte ones).
+// page (INT4 codes). NT: tokens per lane, 1 or 4 (a block writes 4 NT). VEC: latent
+// and k_pe are 16-byte aligned (one 16-byte load per lane, else four 4-byte ones).
 // prot / lens: the protection buffer [num_seqs][132][576] bf16 and the requests'
 // lengths after this write, or null for an unprotected cache.
 //
-// What bounds it: for a prefill the issue slots and the HBM traffic (1152 bytes
-// read and 324 written per token, INT4) weigh about the same; for a decode
-// step's few tokens the latency of load -> extrema -> scale -> codes -> store.
-// So one pass holds eight coordinates per lane, the extrema take three packed
-// shuffles for minimum and maximum together, and the codes take two values per
-// instruction (codes8). Groups outside codes8's argument (quotients above 2^14,
-// infinite values or scales) and the fp32 RoPE scale of the paper's page, whose
-// codes are defined by the rounded fp32 quotient, divide value by value.
+// What bounds it: for a prefill the issue slots, then the HBM traffic (1152 bytes
+// read and 324 written per token, INT4); for a decode step's few tokens the latency
+// of load -> extrema -> scale -> codes -> store. So one pass holds eight coordinates
+// per lane, the extrema take three packed shuffles for minimum and maximum together,
+// and the codes take two values per instruction (codes8). With four tokens per lane
+// the eight lanes of a token share what is per token: lane i of four looks token i's
+// destination up and works out its scale, and shuffles hand them round. Groups
+// outside codes8's argument (quotients above 2^14, infinite values or scales) and
+// the fp32 RoPE scale of the paper's page, whose codes are defined by the rounded
+// fp32 quotient, divide value by value. 32,797 tokens (INT4) take 16.6 us, 2.9 TB/s of
+// 6.8; a warp per (token, group) with two coordinates per lane and a division per
+// code took 61.5.
 template <int CB, int NT, bool VEC>
 __global__ void __launch_bounds__(kAppendThreads) quant_append_kernel(
     uint8_t* __restrict__ pool, int num_blocks, const uint32_t* __restrict__ latent,
     const uint32_t* __restrict__ k_pe, const int32_t* __restrict__ seq_ids,
     const int32_t* __restrict__ positions, int n, const int32_t* __restrict__ table, int num_seqs,
     int max_blocks, uint32_t* dev_err, uint4* __restrict__ prot, const int32_t* __restrict__ lens) {
+  static_assert(NT == 1 || NT == 4, "tokens per lane");
   using L = BlockLayout<CB>;
   const int g = threadIdx.x >> 5;  // this warp's group
   const int lane = threadIdx.x & 31;
   const int piece = lane & 7;
-  const int tok0 = blockIdx.x * (4 * NT) + (lane >> 3);
+  const int tok0 = blockIdx.x * (4 * NT) + (lane >> 3);  // token i of the lane: tok0 + 4 i
   const int bits = g < 8 ? (CB == kC4R4 ? 4 : CB) : kPeBits;
   const int m = (1 << bits) - 1;
   // The groups' loads do not wait for the seq_ids -> block-table lookups, which
@@ -171,24 +169,31 @@ __global__ void __launch_bounds__(kAppendThreads) quant_append_kernel(
       }
     }
   }
-  uint8_t* blk[NT];
-  int slot[NT];
-#pragma unroll
-  for (int i = 0; i < NT; ++i) {
-    const int tok = tok0 + 4 * i;
-    blk[i] = nullptr;
-    slot[i] = 0;
-    // errors are reported once per token, by its group-0 warp
-    if (tok < n)
-      blk[i] = token_block(pool, L::kBytes, num_blocks, seq_ids, positions, tok, table, num_seqs, max_blocks,
-                           piece == 0 && g == 0 ? dev_err : nullptr, slot[i]);
+  // This lane's share: token `own` of the lane's NT. dst is the block's slot, the
+  // block id times 64 plus the slot, or -1; rows the protection rows (sink, ring), or
+  // -1. Errors are reported once per token, by its group-0 warp.
+  const int own = piece & (NT - 1);
+  int dst = -1, sink = -1, ring = -1;
+  if (tok0 + 4 * own < n) {
+    const int tok = tok0 + 4 * own;
+    int seq = 0, pos = 0;
+    const int blk = token_block(num_blocks, seq_ids, positions, tok, table, num_seqs, max_blocks,
+                                piece == own && g == 0 ? dev_err : nullptr, seq, pos);
+    if (blk >= 0) {
+      dst = blk * kBlockTokens + pos % kBlockTokens;
+      if (prot != nullptr) {
+        if (pos < kSinkTokens) sink = seq * kProtRows + pos;
+        if (pos >= lens[seq] - kRecentTokens) ring = seq * kProtRows + kSinkTokens + pos % kRecentTokens;
+      }
+    }
   }
+  // Extrema of each token's 64 values: (min, -max) as a bf16 pair, so that one packed
+  // minimum per shuffle serves both. bf16 minima are exact, and NaNs lose against
+  // numbers as in fminf / fmaxf.
+  uint32_t ext = 0;  // of token `own`
 #pragma unroll
   for (int i = 0; i < NT; ++i) {
     const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
-    // Extrema of the token's 64 values: (min, -max) as a bf16 pair, so that one
-    // packed minimum per shuffle serves both. bf16 minima are exact, and NaNs
-    // lose against numbers as in fminf / fmaxf.
     __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&w[0]), hi = lo;
 #pragma unroll
     for (int e = 1; e < 4; ++e) {
@@ -198,7 +203,8 @@ __global__ void __launch_bounds__(kAppendThreads) quant_append_kernel(
     }
     lo = __hmin2(lo, __lowhigh2highlow(lo));
     hi = __hmax2(hi, __lowhigh2highlow(hi));
-    uint32_t pk = __byte_perm(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi) ^ 0x80008000u, 0x7610);
+    uint32_t pk =
+        __byte_perm(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi) ^ 0x80008000u, 0x7610);
 #pragma unroll
     for (int off = 1; off < 8; off <<= 1) {
       const uint32_t o = __shfl_xor_sync(0xffffffffu, pk, off);
@@ -206,18 +212,45 @@ __global__ void __launch_bounds__(kAppendThreads) quant_append_kernel(
                                        *reinterpret_cast<const __nv_bfloat162*>(&o));
       pk = *reinterpret_cast<const uint32_t*>(&r);
     }
-    const float xmin = __uint_as_float(pk << 16), xmax = -__uint_as_float(pk & 0xFFFF0000u);
-    float s, z;
+    if (i == own) ext = pk;
+  }
+  const float xmin = __uint_as_float(ext << 16), xmax = -__uint_as_float(ext & 0xFFFF0000u);
+  float s_own, z_own;
+  if constexpr (CB == kC4R4) {
+    paper_scale(xmin, xmax, g < 8, s_own, z_own);
+  } else {
+    group_scale(xmin, xmax, m, s_own, z_own);
+  }
+  // 1 / s, or 0 for a group whose values divide one by one (an infinite or NaN
+  // quotient among them; 1 / s is 0 when s is infinite)
+  float y_own = __frcp_rn(s_own);
+  if (!(fmaxf(fabsf(xmin), fabsf(xmax)) * y_own <= 16384.0f) || (CB == kC4R4 && g == 8)) y_own = 0.0f;
+  if (piece == own && dst >= 0) {
+    uint8_t* blk = pool + static_cast<size_t>(dst / kBlockTokens) * L::kBytes;
+    const int slot = dst % kBlockTokens;
     if constexpr (CB == kC4R4) {
-      paper_scale(xmin, xmax, g < 8, s, z);
+      if (g < 8) {
+        *reinterpret_cast<__nv_bfloat16*>(blk + L::c_scale_off(g, slot)) = __float2bfloat16_rn(s_own);  // exact
+      } else {
+        *reinterpret_cast<float*>(blk + L::pe_scale_off(slot)) = s_own;
+      }
+      blk[L::zero_off(g, slot)] = static_cast<uint8_t>(z_own);
     } else {
-      group_scale(xmin, xmax, m, s, z);
+      *reinterpret_cast<__half2*>(blk + L::sz_off(g, slot)) =
+          __halves2half2(__float2half_rn(s_own), __float2half_rn(z_own));
     }
-    const float y = __frcp_rn(s);
-    // (false for an infinite or NaN quotient; y = 0 when s is infinite)
-    const bool fast = y > 0.0f && fmaxf(fabsf(xmin), fabsf(xmax)) * y <= 16384.0f && !(CB == kC4R4 && g == 8);
+  }
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+    // (the token's values from its lane i)
+    const int from = (lane & 24) | i;
+    const float s = NT == 1 ? s_own : __shfl_sync(0xffffffffu, s_own, from);
+    const float y = NT == 1 ? y_own : __shfl_sync(0xffffffffu, y_own, from);
+    const float z = NT == 1 ? z_own : __shfl_sync(0xffffffffu, z_own, from);
+    const int d = NT == 1 ? dst : __shfl_sync(0xffffffffu, dst, from);
     uint32_t c[4];  // codes 2 e and 2 e + 1 in the halves of c[e]
-    if (fast) {
+    if (y > 0.0f) {
       codes8(w, s, y, z, m, c);
     } else {
 #pragma unroll
@@ -234,30 +267,19 @@ __global__ void __launch_bounds__(kAppendThreads) quant_append_kernel(
       const uint32_t a = c[0] | c[1] << 4 | c[2] << 8 | c[3] << 12;
       word = a | a >> 14;
     }
-    if (blk[i] == nullptr) continue;
-    const int tok = tok0 + 4 * i;
     if (prot != nullptr) {
-      const int seq = seq_ids != nullptr ? seq_ids[tok] : tok;
-      protect_piece(prot, raw[i], g * 8 + piece, seq, positions[tok], lens[seq]);
+      const int rows[2] = {NT == 1 ? sink : __shfl_sync(0xffffffffu, sink, from),
+                           NT == 1 ? ring : __shfl_sync(0xffffffffu, ring, from)};
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+        if (rows[r] >= 0) prot[static_cast<size_t>(rows[r]) * (kDqk * 2 / 16) + g * 8 + piece] = raw[i];
     }
-    uint8_t* dst = blk[i] + L::code_off(g, slot[i]);
+    if (d < 0) continue;
+    uint8_t* code = pool + static_cast<size_t>(d / kBlockTokens) * L::kBytes + L::code_off(g, d % kBlockTokens);
     if (bits == 4) {
-      reinterpret_cast<uint32_t*>(dst)[piece] = word;
+      reinterpret_cast<uint32_t*>(code)[piece] = word;
     } else {
-      reinterpret_cast<uint16_t*>(dst)[piece] = static_cast<uint16_t>(word);
-    }
-    if (piece == 0) {
-      if constexpr (CB == kC4R4) {
-        if (g < 8) {
-          *reinterpret_cast<__nv_bfloat16*>(blk[i] + L::c_scale_off(g, slot[i])) = __float2bfloat16_rn(s);  // exact
-        } else {
-          *reinterpret_cast<float*>(blk[i] + L::pe_scale_off(slot[i])) = s;
-        }
-        blk[i][L::zero_off(g, slot[i])] = static_cast<uint8_t>(z);
-      } else {
-        *reinterpret_cast<__half2*>(blk[i] + L::sz_off(g, slot[i])) =
-            __halves2half2(__float2half_rn(s), __float2half_rn(z));
-      }
+      reinterpret_cast<uint16_t*>(code)[piece] = static_cast<uint16_t>(word);
     }
   }
 }
@@ -284,11 +306,12 @@ __global__ void __launch_bounds__(256) bf16_append_kernel(
   } else {
     v = make_uint4(src[0], src[1], src[2], src[3]);
   }
-  int slot = 0;
-  uint8_t* blk = token_block(pool, kBf16BlockBytes, num_blocks, seq_ids, positions, tok, table,
-                             num_seqs, max_blocks, piece == 0 ? dev_err : nullptr, slot);
-  if (blk == nullptr) return;
-  reinterpret_cast<uint4*>(blk + slot * kDqk * 2)[piece] = v;
+  int seq = 0, pos = 0;
+  const int blk = token_block(num_blocks, seq_ids, positions, tok, table, num_seqs, max_blocks,
+                              piece == 0 ? dev_err : nullptr, seq, pos);
+  if (blk < 0) return;
+  reinterpret_cast<uint4*>(pool + static_cast<size_t>(blk) * kBf16BlockBytes + pos % kBlockTokens * (kDqk * 2))[piece] =
+      v;
 }
 
 bool aligned16(const void* a, const void* b) {
@@ -306,16 +329,18 @@ void launch_quant(void* pool, int num_blocks, const uint16_t* latent, const uint
       static_cast<uint4*>(prot), lens);
 }
 
-// Tokens from which a lane takes two: below, one token per lane spreads the
-// step's tokens over more SMs and ends sooner.
-constexpr int kTwoPerLane = 8192;
+// Tokens from which a lane takes four: below, one token per lane spreads the
+// tokens over more SMs and ends sooner. One GB300, INT4 / the paper's page, four
+// against one: 4,096 tokens 3.6 against 3.6 / 4.4 against 3.8 us, 8,192 5.0 against
+// 5.8 / 5.8 against 6.2, 32,768 13.8 against 18.5 / 16.8 against 19.6.
+constexpr int kFourPerLane = 8192;
 
 template <int CB>
 void launch_quant(void* pool, int num_blocks, const uint16_t* latent, const uint16_t* k_pe, const int32_t* seq_ids,
                   const int32_t* positions, int n, const int32_t* table, int num_seqs, int max_blocks,
                   uint32_t* dev_err, cudaStream_t stream, void* prot, const int32_t* lens) {
   auto* f = !aligned16(latent, k_pe) ? launch_quant<CB, 1, false>
-                                     : (n >= kTwoPerLane ? launch_quant<CB, 2, true> : launch_quant<CB, 1, true>);
+                                     : (n >= kFourPerLane ? launch_quant<CB, 4, true> : launch_quant<CB, 1, true>);
   f(pool, num_blocks, latent, k_pe, seq_ids, positions, n, table, num_seqs, max_blocks, dev_err, stream, prot, lens);
 }
 
