@@ -13,6 +13,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "ptx.cuh"
 
 namespace qmla {
 namespace {
@@ -146,6 +147,9 @@ __global__ void __launch_bounds__(kAppendThreads) quant_append_kernel(
     int max_blocks, uint32_t* dev_err, uint4* __restrict__ prot, const int32_t* __restrict__ lens) {
   static_assert(NT == 1 || NT == 4, "tokens per lane");
   using L = BlockLayout<CB>;
+  // The decode's prep kernel may start meanwhile (it does not read the cache, and
+  // does not end before this kernel has).
+  griddep_launch_dependents();
   const int g = threadIdx.x >> 5;  // this warp's group
   const int lane = threadIdx.x & 31;
   const int piece = lane & 7;
@@ -294,6 +298,7 @@ __global__ void __launch_bounds__(256) bf16_append_kernel(
     const int32_t* __restrict__ positions, int n, const int32_t* __restrict__ table, int num_seqs,
     int max_blocks, uint32_t* dev_err) {
   constexpr int kPieces = kDqk * 2 / 16;
+  griddep_launch_dependents();  // as in quant_append_kernel
   const long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int tok = static_cast<int>(idx / kPieces);
   const int piece = static_cast<int>(idx - static_cast<long long>(tok) * kPieces);
