@@ -103,18 +103,21 @@ def lib():
     return L
 
 
+# Addresses and stream handles travel as plain integers (the argtypes convert them),
+# and the stream comes straight from the raw handle: a call's marshalling costs about
+# as much as a launch, and small decode steps are bound by it.
 def _ptr(t: torch.Tensor | None):
     if t is None:
         return None
     if not t.is_contiguous():
         raise ValueError("tensors must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _check(fn: str, st: int) -> None:
@@ -143,10 +146,10 @@ def quant_append(pool: torch.Tensor, c_bits: int, latent: torch.Tensor, k_pe: to
                  dev_err: torch.Tensor, stream=None) -> None:
     """qmla_quant_append: pool uint8 [num_blocks, block_bytes]; latent bf16 [n,512];
     k_pe bf16 [n,64]; seq_ids/positions int32 [n]; block_table int32 [S, max_blocks]."""
-    n = latent.shape[0]
-    st = lib().qmla_quant_append(_ptr(pool), c_bits, pool.shape[0], _ptr(latent), _ptr(k_pe), _ptr(seq_ids),
-                                 _ptr(positions), n, _ptr(block_table), block_table.shape[0],
-                                 block_table.shape[1], _ptr(dev_err), _stream(stream))
+    n = latent.size(0)
+    st = lib().qmla_quant_append(_ptr(pool), c_bits, pool.size(0), _ptr(latent), _ptr(k_pe), _ptr(seq_ids),
+                                 _ptr(positions), n, _ptr(block_table), block_table.size(0),
+                                 block_table.size(1), _ptr(dev_err), _stream(stream))
     _check("qmla_quant_append", st)
 
 
@@ -159,19 +162,19 @@ def quant_append_protected(pool: torch.Tensor, c_bits: int, latent: torch.Tensor
                            seq_lens: torch.Tensor, prot: torch.Tensor, dev_err: torch.Tensor, stream=None) -> None:
     """qmla_quant_append_protected: quant_append plus the sink/recent bf16 rows;
     seq_lens int32 [S] = lengths after this call; prot [S, 132, 576] bf16."""
-    n = latent.shape[0]
-    st = lib().qmla_quant_append_protected(_ptr(pool), c_bits, pool.shape[0], _ptr(latent), _ptr(k_pe),
+    n = latent.size(0)
+    st = lib().qmla_quant_append_protected(_ptr(pool), c_bits, pool.size(0), _ptr(latent), _ptr(k_pe),
                                            _ptr(seq_ids), _ptr(positions), n, _ptr(block_table),
-                                           block_table.shape[0], block_table.shape[1], _ptr(seq_lens), _ptr(prot),
+                                           block_table.size(0), block_table.size(1), _ptr(seq_lens), _ptr(prot),
                                            _ptr(dev_err), _stream(stream))
     _check("qmla_quant_append_protected", st)
 
 
 def bf16_append(pool: torch.Tensor, latent: torch.Tensor, k_pe: torch.Tensor, seq_ids: torch.Tensor | None,
                 positions: torch.Tensor, block_table: torch.Tensor, dev_err: torch.Tensor, stream=None) -> None:
-    n = latent.shape[0]
-    st = lib().qmla_bf16_append(_ptr(pool), pool.shape[0], _ptr(latent), _ptr(k_pe), _ptr(seq_ids),
-                                _ptr(positions), n, _ptr(block_table), block_table.shape[0], block_table.shape[1],
+    n = latent.size(0)
+    st = lib().qmla_bf16_append(_ptr(pool), pool.size(0), _ptr(latent), _ptr(k_pe), _ptr(seq_ids),
+                                _ptr(positions), n, _ptr(block_table), block_table.size(0), block_table.size(1),
                                 _ptr(dev_err), _stream(stream))
     _check("qmla_bf16_append", st)
 
@@ -180,10 +183,10 @@ def mla_decode(pool: torch.Tensor, c_bits: int, q_latent: torch.Tensor, q_pe: to
                block_table: torch.Tensor, seq_lens: torch.Tensor, softmax_scale: float, out: torch.Tensor,
                lse: torch.Tensor | None, workspace: torch.Tensor, dev_err: torch.Tensor, stream=None) -> None:
     """qmla_mla_decode: q_latent bf16 [B,H,512], q_pe bf16 [B,H,64], out f32 [B,H,512], lse f32 [B,H]."""
-    B, H = q_latent.shape[0], q_latent.shape[1]
-    st = lib().qmla_mla_decode(_ptr(pool), c_bits, pool.shape[0], _ptr(q_latent), _ptr(q_pe), B, H,
-                               _ptr(block_table), block_table.shape[1], _ptr(seq_lens), float(softmax_scale),
-                               _ptr(out), _ptr(lse), _ptr(workspace), workspace.numel() * workspace.element_size(),
+    B, H = q_latent.size(0), q_latent.size(1)
+    st = lib().qmla_mla_decode(_ptr(pool), c_bits, pool.size(0), _ptr(q_latent), _ptr(q_pe), B, H,
+                               _ptr(block_table), block_table.size(1), _ptr(seq_lens), float(softmax_scale),
+                               _ptr(out), _ptr(lse), _ptr(workspace), workspace.nbytes,
                                _ptr(dev_err), _stream(stream))
     _check("qmla_mla_decode", st)
 
@@ -193,11 +196,11 @@ def mla_decode_protected(pool: torch.Tensor, c_bits: int, q_latent: torch.Tensor
                          out: torch.Tensor, lse: torch.Tensor | None, workspace: torch.Tensor, dev_err: torch.Tensor,
                          stream=None) -> None:
     """qmla_mla_decode_protected: mla_decode with sink4/local128 bf16 rows from prot [B, 132, 576]."""
-    B, H = q_latent.shape[0], q_latent.shape[1]
-    st = lib().qmla_mla_decode_protected(_ptr(pool), c_bits, pool.shape[0], _ptr(q_latent), _ptr(q_pe), B, H,
-                                         _ptr(block_table), block_table.shape[1], _ptr(seq_lens), _ptr(prot),
+    B, H = q_latent.size(0), q_latent.size(1)
+    st = lib().qmla_mla_decode_protected(_ptr(pool), c_bits, pool.size(0), _ptr(q_latent), _ptr(q_pe), B, H,
+                                         _ptr(block_table), block_table.size(1), _ptr(seq_lens), _ptr(prot),
                                          float(softmax_scale), _ptr(out), _ptr(lse), _ptr(workspace),
-                                         workspace.numel() * workspace.element_size(), _ptr(dev_err),
+                                         workspace.nbytes, _ptr(dev_err),
                                          _stream(stream))
     _check("qmla_mla_decode_protected", st)
 
@@ -208,11 +211,11 @@ def mla_decode_multi(pool: torch.Tensor, c_bits: int, q_latent: torch.Tensor, q_
                      prot: torch.Tensor | None = None, stream=None) -> None:
     """qmla_mla_decode_multi: q_latent bf16 [B,T,H,512], q_pe bf16 [B,T,H,64],
     out f32 [B,T,H,512], lse f32 [B,T,H]; workspace for B x (T*H) heads."""
-    B, T, H = q_latent.shape[0], q_latent.shape[1], q_latent.shape[2]
-    st = lib().qmla_mla_decode_multi(_ptr(pool), c_bits, pool.shape[0], _ptr(q_latent), _ptr(q_pe), B, T, H,
-                                     _ptr(block_table), block_table.shape[1], _ptr(seq_lens), _ptr(prot),
+    B, T, H = q_latent.size(0), q_latent.size(1), q_latent.size(2)
+    st = lib().qmla_mla_decode_multi(_ptr(pool), c_bits, pool.size(0), _ptr(q_latent), _ptr(q_pe), B, T, H,
+                                     _ptr(block_table), block_table.size(1), _ptr(seq_lens), _ptr(prot),
                                      float(softmax_scale), _ptr(out), _ptr(lse), _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _ptr(dev_err), _stream(stream))
+                                     workspace.nbytes, _ptr(dev_err), _stream(stream))
     _check("qmla_mla_decode_multi", st)
 
 
@@ -225,8 +228,8 @@ def debug_tile(pool: torch.Tensor, cache_kind: int, block_table: torch.Tensor, s
                stream=None) -> None:
     """qmla_debug_tile: tile j of sequence b as the decode kernel builds it, into
     tile [128, 576] (fp16 or int16)."""
-    st = lib().qmla_debug_tile(_ptr(pool), cache_kind, pool.shape[0], _ptr(block_table), block_table.shape[1],
-                               _ptr(seq_lens), block_table.shape[0], b, j, _ptr(prot), _ptr(tile), _ptr(dev_err),
+    st = lib().qmla_debug_tile(_ptr(pool), cache_kind, pool.size(0), _ptr(block_table), block_table.size(1),
+                               _ptr(seq_lens), block_table.size(0), b, j, _ptr(prot), _ptr(tile), _ptr(dev_err),
                                _stream(stream))
     _check("qmla_debug_tile", st)
 
@@ -249,10 +252,10 @@ def quant_append_c4r4(pool: torch.Tensor, latent: torch.Tensor, k_pe: torch.Tens
                       seq_lens: torch.Tensor | None = None, prot: torch.Tensor | None = None, stream=None) -> None:
     """qmla_quant_append_c4r4: pages of the paper's format; with prot (and
     seq_lens = lengths after this call) also the sink/recent bf16 rows."""
-    n = latent.shape[0]
-    st = lib().qmla_quant_append_c4r4(_ptr(pool), pool.shape[0], _ptr(latent), _ptr(k_pe), _ptr(seq_ids),
-                                      _ptr(positions), n, _ptr(block_table), block_table.shape[0],
-                                      block_table.shape[1], _ptr(seq_lens), _ptr(prot), _ptr(dev_err),
+    n = latent.size(0)
+    st = lib().qmla_quant_append_c4r4(_ptr(pool), pool.size(0), _ptr(latent), _ptr(k_pe), _ptr(seq_ids),
+                                      _ptr(positions), n, _ptr(block_table), block_table.size(0),
+                                      block_table.size(1), _ptr(seq_lens), _ptr(prot), _ptr(dev_err),
                                       _stream(stream))
     _check("qmla_quant_append_c4r4", st)
 
@@ -263,22 +266,22 @@ def mla_decode_c4r4(pool: torch.Tensor, q_latent: torch.Tensor, q_pe: torch.Tens
                     stream=None) -> None:
     """qmla_mla_decode_c4r4: mla_decode over pages of the paper's format, with
     sink4/local128 protection when prot [B, 132, 576] is given."""
-    B, H = q_latent.shape[0], q_latent.shape[1]
-    st = lib().qmla_mla_decode_c4r4(_ptr(pool), pool.shape[0], _ptr(q_latent), _ptr(q_pe), B, H, _ptr(block_table),
-                                    block_table.shape[1], _ptr(seq_lens), _ptr(prot), float(softmax_scale),
+    B, H = q_latent.size(0), q_latent.size(1)
+    st = lib().qmla_mla_decode_c4r4(_ptr(pool), pool.size(0), _ptr(q_latent), _ptr(q_pe), B, H, _ptr(block_table),
+                                    block_table.size(1), _ptr(seq_lens), _ptr(prot), float(softmax_scale),
                                     _ptr(out), _ptr(lse), _ptr(workspace),
-                                    workspace.numel() * workspace.element_size(), _ptr(dev_err), _stream(stream))
+                                    workspace.nbytes, _ptr(dev_err), _stream(stream))
     _check("qmla_mla_decode_c4r4", st)
 
 
 def mla_decode_bf16cache(pool: torch.Tensor, q_latent: torch.Tensor, q_pe: torch.Tensor, block_table: torch.Tensor,
                          seq_lens: torch.Tensor, softmax_scale: float, out: torch.Tensor, lse: torch.Tensor | None,
                          workspace: torch.Tensor, dev_err: torch.Tensor, stream=None) -> None:
-    B, H = q_latent.shape[0], q_latent.shape[1]
-    st = lib().qmla_mla_decode_bf16cache(_ptr(pool), pool.shape[0], _ptr(q_latent), _ptr(q_pe), B, H,
-                                         _ptr(block_table), block_table.shape[1], _ptr(seq_lens),
+    B, H = q_latent.size(0), q_latent.size(1)
+    st = lib().qmla_mla_decode_bf16cache(_ptr(pool), pool.size(0), _ptr(q_latent), _ptr(q_pe), B, H,
+                                         _ptr(block_table), block_table.size(1), _ptr(seq_lens),
                                          float(softmax_scale), _ptr(out), _ptr(lse), _ptr(workspace),
-                                         workspace.numel() * workspace.element_size(), _ptr(dev_err),
+                                         workspace.nbytes, _ptr(dev_err),
                                          _stream(stream))
     _check("qmla_mla_decode_bf16cache", st)
 
@@ -288,9 +291,9 @@ def mla_decode_static(pool: torch.Tensor, c_bits: int, q_latent: torch.Tensor, q
                       lse: torch.Tensor | None, dev_err: torch.Tensor, stream=None) -> None:
     """qmla_mla_decode_static: qmla_mla_decode for callers that cannot allocate a
     workspace; uses the library's fixed device scratch (see include/qmla.h)."""
-    B, H = q_latent.shape[0], q_latent.shape[1]
-    st = lib().qmla_mla_decode_static(_ptr(pool), c_bits, pool.shape[0], _ptr(q_latent), _ptr(q_pe), B, H,
-                                      _ptr(block_table), block_table.shape[1], _ptr(seq_lens),
+    B, H = q_latent.size(0), q_latent.size(1)
+    st = lib().qmla_mla_decode_static(_ptr(pool), c_bits, pool.size(0), _ptr(q_latent), _ptr(q_pe), B, H,
+                                      _ptr(block_table), block_table.size(1), _ptr(seq_lens),
                                       float(softmax_scale), _ptr(out), _ptr(lse), _ptr(dev_err), _stream(stream))
     _check("qmla_mla_decode_static", st)
 
@@ -307,15 +310,15 @@ def mla_decode_ex(pool: torch.Tensor, cache_kind, q_latent: torch.Tensor, q_pe: 
     [B,T,H,512]; events = (before_main, after_main) torch.cuda.Event pair (already
     recorded once, so that they exist) to record around this call's main kernel."""
     if q_latent.dim() == 3:
-        B, T, H = q_latent.shape[0], 1, q_latent.shape[1]
+        B, T, H = q_latent.size(0), 1, q_latent.size(1)
     else:
-        B, T, H = q_latent.shape[0], q_latent.shape[1], q_latent.shape[2]
+        B, T, H = q_latent.size(0), q_latent.size(1), q_latent.size(2)
     d = DecodeDesc()
-    d.pool, d.cache_kind, d.num_blocks = _ptr(pool), CACHE_KINDS[cache_kind], pool.shape[0]
+    d.pool, d.cache_kind, d.num_blocks = _ptr(pool), CACHE_KINDS[cache_kind], pool.size(0)
     d.q_latent, d.q_pe, d.batch, d.q_tokens, d.heads = _ptr(q_latent), _ptr(q_pe), B, T, H
-    d.block_table, d.max_blocks, d.seq_lens = _ptr(block_table), block_table.shape[1], _ptr(seq_lens)
+    d.block_table, d.max_blocks, d.seq_lens = _ptr(block_table), block_table.size(1), _ptr(seq_lens)
     d.prot, d.softmax_scale, d.out, d.lse = _ptr(prot), float(softmax_scale), _ptr(out), _ptr(lse)
-    d.workspace, d.workspace_bytes = _ptr(workspace), workspace.numel() * workspace.element_size()
+    d.workspace, d.workspace_bytes = _ptr(workspace), workspace.nbytes
     d.dev_err = _ptr(dev_err)
     if events is not None:
         d.ev_before_main = ctypes.c_void_p(events[0].cuda_event) if events[0] is not None else None
