@@ -181,7 +181,7 @@ def profile_traffic(kernel_file_hash: str, workload: str, bf16: bool = False, pr
 
 
 # The sources decode_main is compiled from (its translation unit and headers).
-DECODE_MAIN_SOURCES = ("common.cuh", "decode.cu", "kernels.h", "ptx.cuh")
+DECODE_MAIN_SOURCES = ("common.cuh", "decode.cu", "decode_common.cuh", "decode_pair.cu", "kernels.h", "ptx.cuh")
 
 
 def decode_cu_hash() -> str:
