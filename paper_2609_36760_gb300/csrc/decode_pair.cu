@@ -443,7 +443,7 @@ __device__ void pair_softmax(const Params& p, PairSched sc, uint32_t smem, PairC
   };
   // Settles the last tile (real tile v - 1, n - 1 among all) once every warp has given
   // its P: where one of them had a weight above 2^8, the reference is raised and P
-  // rewritten (the issuer waits for p_fixed). Done at the next tile, so that nobody
+  // rewritten (PV waits for p_fixed). Done at the next tile, so that nobody
   // waits for the other warps; until then its scores stay.
   bool due = false;
   int vis_due = 0;
@@ -663,16 +663,21 @@ __device__ void pair_mma(const Params& p, const PairSched& sc, uint8_t* sm, uint
     if (sp.live) {
       const bool first = sp.seg_first();
       const uint32_t st = v & 1u, ph = (v >> 1) & 1u;
-      if (mbar_test(&ctl.p_full[st], ph) && mbar_test(&ctl.v_full[st], ph) &&
-          (!first || pseg == 0 || mbar_test(&ctl.o_free, (pseg - 1) & 1u))) {
+      bool ready = mbar_test(&ctl.p_full[st], ph) && mbar_test(&ctl.v_full[st], ph) &&
+                   (!first || pseg == 0 || mbar_test(&ctl.o_free, (pseg - 1) & 1u));
+      // A rewritten P is waited for by passing on to the QK below: the softmax settles a
+      // tile when it has the next one's scores, which may not have been issued yet.
+      bool fix[2] = {false, false};
+      if (ready) {
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          if (ok && *reinterpret_cast<volatile uint32_t*>(&ctl.raised[r][st]) == v + 1) {
-            ok = pwait(&ctl.p_fixed[r], fixes[r] & 1u, ctl, kSiteMmaPFull, p.dev_err);
-            ++fixes[r];
-          }
+          fix[r] = *reinterpret_cast<volatile uint32_t*>(&ctl.raised[r][st]) == v + 1;
+          ready = ready && (!fix[r] || mbar_test(&ctl.p_fixed[r], fixes[r] & 1u));
         }
-        if (!ok) break;
+      }
+      if (ready) {
+        fixes[0] += fix[0] ? 1u : 0u;
+        fixes[1] += fix[1] ? 1u : 0u;
         tc_fence_after();
         const uint64_t a1 = pa + ((st * kPTile) >> 4), b1 = vb + ((st * kVStage) >> 4);
         const uint32_t acc0 = first ? 0u : 1u;
