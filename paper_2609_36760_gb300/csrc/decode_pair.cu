@@ -444,21 +444,26 @@ __device__ void pair_softmax(const Params& p, PairSched sc, uint32_t smem, PairC
   // Settles the last tile (real tile v - 1, n - 1 among all) once every warp has given
   // its P: where one of them had a weight above 2^8, the reference is raised and P
   // rewritten (PV waits for p_fixed). Done at the next tile, so that nobody
-  // waits for the other warps; until then its scores stay.
+  // waits for the other warps; until then its scores stay. The raised reference covers
+  // the whole 128-token tile, as a renewed one does: an even block takes in the odd one
+  // behind it (`next`: its scores are in the following buffer), an odd one the even one
+  // before it, whose scores are therefore released with the odd one's.
   bool due = false;
   int vis_due = 0;
   float l_due = 0.0f;
-  auto settle = [&]() {
+  auto settle = [&](bool odd, bool next) {
     due = false;
     if (!(ok = wwait(&ctl.grp, gph & 1u, ctl, kSiteGrp, p.dev_err))) return false;
     ++gph;
     const uint32_t st = (v - 1) & 1u;
     if (*reinterpret_cast<volatile uint32_t*>(&ctl.over[st]) == v) {
-      const float mx = tmem_scores_max(t_s(n - 1), sl2, vis_due);
+      float mx = tmem_scores_max(t_s(n - 1), sl2, vis_due);
+      if (odd || next)
+        mx = fmaxf(mx, tmem_scores_max(t_s(odd ? n - 2 : n), sl2, odd ? vis_due + kPairTok : vis_due - kPairTok));
       float mo = 0.0f;
       if (!exchange(mx, mo)) return false;
       if (!move_ref(fmaxf(m, fmaxf(mx, mo)), v - 1)) return false;
-      l_due = 0.0f;
+      float l0 = 0.0f, l1 = 0.0f;
 #pragma unroll 1
       for (int c = 0; c < 32; c += 8) {
         uint32_t a[8], b[8], w[4];
@@ -470,16 +475,18 @@ __device__ void pair_softmax(const Params& p, PairSched sc, uint32_t smem, PairC
           const float y0 = __fmaf_rn(__uint_as_float(a[2 * i]) + __uint_as_float(b[2 * i]), sl2, -m);
           const float y1 = __fmaf_rn(__uint_as_float(a[2 * i + 1]) + __uint_as_float(b[2 * i + 1]), sl2, -m);
           w[i] = pack_h2(c + 2 * i < vis_due ? ex2_approx(y0) : 0.0f, c + 2 * i + 1 < vis_due ? ex2_approx(y1) : 0.0f);
-          add_h2(l_due, l_due, w[i]);
+          add_h2(l0, l1, w[i]);
         }
         sts_v4(smem + kPOff + st * kPTile + swz_off(row, half * 4 + c / 8, 128), w[0], w[1], w[2], w[3]);
       }
+      l_due = l0 + l1;
       fence_proxy_async_smem();
       tc_fence_before();
       __syncwarp();
       arrive_leader(lane, pfixed);
     }
-    release_s(n - 1);
+    if (odd) release_s(n - 2);
+    if (!next) release_s(n - 1);
     l += l_due;
     return true;
   };
@@ -533,7 +540,7 @@ __device__ void pair_softmax(const Params& p, PairSched sc, uint32_t smem, PairC
     }
     if (!wait_s(n)) break;
     load_scores(t_s(n), x);
-    if (due && !settle()) break;
+    if (due && !settle(even, !even)) break;
     vis = vis_end - (kPairTok * sc.q + 32 * half);
     if (renew) {
       float mx = scores_max(x, sl2, vis);
@@ -570,7 +577,7 @@ __device__ void pair_softmax(const Params& p, PairSched sc, uint32_t smem, PairC
     if (!sc.seg_last()) continue;
 
     // ---- segment end: out = O / l, or the partial (m, l, o)
-    if (due && !settle()) break;
+    if (due && !settle(!even, false)) break;
     whole = whole && sc.t1 >= sc.pu1;
     float lo = 0.0f;
     if (!exchange(l, lo)) break;

@@ -101,3 +101,35 @@ def test_pair_bad_block_flags_error_and_spares_neighbours():
     assert c.dev_error() == 1
     assert np.isfinite(out).all() and np.isfinite(lse).all()
     assert np.array_equal(out[1], good[1])
+
+
+@pytest.mark.parametrize("kind", ["int4", "int2", "bf16"])
+def test_pair_raises_inside_a_range(kind):
+    # 564 tiles, several per range of the plan; single tokens that exceed the reference by
+    # far more than 2^8 at places of either parity of block, some with most of the sum
+    lengths = (9000, 8000, 9500, 7000)
+    bits = 2 if kind == "int2" else 4
+    w = W.small_workload("r", batch=4, heads=128, lengths=lengths, c_bits=bits, seed=72)
+    c = Case(w, bf16_cache=kind == "bf16")
+    ql, qp = W.queries(w, 0)
+    for b in range(w.batch):
+        lat, kp = c.tokens(b)
+        lat = lat.double() * 0.2
+        for i, at in enumerate(range(170 + 17 * b, lat.shape[0], 450)):
+            q = ql.double()[b, 5 * i % 128]
+            lat[at] = q / q.norm() * lat[at].norm() * (1.2, 1.8, 3.0)[i % 3]
+        c._tok[b] = (lat.to(torch.bfloat16), kp)
+    c.prefill_all()
+    ql = (ql.double() * 12.0).to(torch.bfloat16)
+    out_n, lse_n = c.decode(0, queries=(ql, qp))
+    _widen(c)
+    out_w, lse_w = c.decode(0, queries=(ql, qp))
+    assert c.dev_error() == 0
+    for b in range(w.batch):
+        # the same references, but for the weights of the even blocks of tiles that an odd
+        # block raised: 2^-11 of at most one block's share of the sum
+        assert rel_l2(out_w[b], out_n[b]) <= 2.0 ** -11, b
+        assert np.max(np.abs(lse_w[b] - lse_n[b])) <= 2.0 ** -11 * max(1.0, np.max(np.abs(lse_n[b])))
+        ref, rlse = c.oracle_decode(b, c.prefill[b], 0, fp16_tiles=True, queries=(ql, qp))
+        assert rel_l2(out_w[b], ref) <= 1e-3
+        assert np.max(np.abs(lse_w[b] - rlse)) <= 1e-3 * max(1.0, np.abs(rlse).max())
