@@ -840,18 +840,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) dec
   // prep and the cache writer before it produced.
   griddep_wait();
 
-  PairSched sc;
-  sc.init(p, pair);
+  // (Each role makes its own schedule: one made before the branch, held across the
+  // register split, spilled 244 instead of 60 bytes; 64 x 4,097 tokens, INT4: 120.8 us
+  // instead of 115.1, BF16 168.5 instead of 163.3, INT2 32 x 32,768 386 instead of 368.)
   if (warp < kSoftWarps) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftRegs));
+    PairSched sc;
+    sc.init(p, pair);
     pair_softmax<CB>(p, sc, smem, ctl, tmem, rank, warp, lane, pair);
   } else {
    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
    if (warp < kMmaWarp) {
+    PairSched sc;
+    sc.init(p, pair);
     pair_dequant<CB, PROT>(p, sc, smem, ctl, rank, warp - kSoftWarps, lane);
    } else if (warp > kPrefetchWarp) {
     asm volatile("exit;");
    } else if (elect_one()) {  // the issuers are single threads
+    PairSched sc;
+    sc.init(p, pair);
     if (warp == kMmaWarp) {
       if (rank == 0) {
         pair_mma(p, sc, sm, smem, ctl, tmem);
