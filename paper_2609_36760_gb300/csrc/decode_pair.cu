@@ -18,8 +18,8 @@
 // and 64 rows of each CTA, beside the softmax. What bounds the kernel now is the softmax
 // warps' turn, about 3.1k cycles per 64-token tile, most of it waits on shared memory and
 // TMEM behind the other warps' bursts. One GB300, a decode step of 64 sequences x 128
-// heads x 4,097 tokens, decode_main / this: INT4 127.7 / 120.7 us, the paper's page with
-// protection 174.2 / 141.1, BF16 237.4 / 168.2; INT2, 32 x 32,768 tokens: 396.7 / 374.5.
+// heads x 4,097 tokens, decode_main / this: INT4 129.0 / 115.1 us, the paper's page with
+// protection 174.2 / 138.1, BF16 237.4 / 163.3; INT2, 32 x 32,768 tokens: 395.5 / 368.2.
 // (A second softmax group, one per alternate tile, was slower: 152 us on the INT4 step,
 // its warps' extra waits and registers cost more than their overlap gave.)
 //
@@ -843,6 +843,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) dec
   // (Each role makes its own schedule: one made before the branch, held across the
   // register split, spilled 244 instead of 60 bytes; 64 x 4,097 tokens, INT4: 120.8 us
   // instead of 115.1, BF16 168.5 instead of 163.3, INT2 32 x 32,768 386 instead of 368.)
+  // (Each role makes its own schedule: one made before the branch and held across the
+  // register split spilled up to 244 bytes; the INT4 step then took 120.8 us.)
   if (warp < kSoftWarps) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftRegs));
     PairSched sc;
