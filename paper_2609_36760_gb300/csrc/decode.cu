@@ -30,6 +30,8 @@
 //                  chunk is overwritten only after the PV that reads it commits.
 //                  At a segment end the softmax warps write the final output, or
 //                  an unnormalised partial (m, l, o) when the unit is split.
+//                  (decode_pair takes its place for even numbers of 64-head groups
+//                  over longer contexts, see use_pair.)
 //   combine_kernel merges the partials of split units with
 //                  m = max m_j, l = sum e^(m_j - m) l_j, O = sum e^(m_j - m) o_j / l
 //                  (combine_wide_kernel for a few long units).
@@ -1297,12 +1299,12 @@ cudaError_t launch_hg(int hg, bool pair, const Params& prm, cudaStream_t stream,
 // fixed part (the reference tiles above all). The pair gains most where decode_main's
 // workers have most to do per row: measured on one GB300 (decode alone, 128 heads,
 // decode_main against the pair, us; in brackets the tiles per SM):
-//   INT4            32 x 4,000 (13) 72.6 / 74.2   4 x 60,000 (25) 103.5 /  90.3
-//   INT2            32 x 4,000 (13) 72.7 / 77.5   4 x 60,000 (25) 103.5 /  96.8
-//   the paper's page 16 x 4,000 (7) 56.9 / 58.8   64 x 2,000 (13)  86.2 /  84.6
-//   INT4, protected  4 x 4,000 (1.7) 31.3 / 26.4  32 x 4,000 (13)  88.2 /  79.6
-//   page, protected  4 x 4,000 (1.7) 31.6 / 26.6  32 x 4,000 (13)  96.1 /  85.5
-//   BF16 cache       4 x 4,000 (1.7) 32.8 / 28.0  32 x 4,000 (13) 129.3 /  98.1
+//   INT4             16 x 4,000 (7) 51.9 / 53.0   32 x 4,000 (13) 72.6 /  70.4
+//   INT2            32 x 4,000 (13) 72.8 / 76.9   64 x 4,097 (28) 124.3 / 122.6
+//   the paper's page 16 x 4,000 (7) 57.3 / 58.3   64 x 2,000 (13)  86.0 /  82.8
+//   INT4, protected  4 x 4,000 (1.7) 30.9 / 26.1  32 x 4,000 (13)  87.9 /  78.5
+//   page, protected  4 x 4,000 (1.7) 31.5 / 26.5  32 x 4,000 (13)  96.3 /  84.9
+//   BF16 cache       4 x 4,000 (1.7) 32.7 / 27.4  32 x 4,000 (13) 128.4 /  95.0
 bool use_pair(const DecodeArgs& a) {
 #ifdef QMLA_TRACE_BUILD
   return false;  // the timeline is decode_main's
@@ -1311,7 +1313,7 @@ bool use_pair(const DecodeArgs& a) {
   if (groups % 2 != 0 || a.grid < 2) return false;
   const long long most_tiles = static_cast<long long>(a.batch) * groups * ((static_cast<long long>(a.max_blocks) + 1) / 2);
   const bool heavy_rows = a.cache_kind == 16 || a.prot != nullptr;
-  const double per_sm = heavy_rows ? 1.5 : (a.cache_kind == kC4R4 ? 10.0 : 18.0);
+  const double per_sm = heavy_rows ? 1.5 : (a.cache_kind == kC4R4 ? 10.0 : a.cache_kind == 4 ? 12.0 : 18.0);
   return static_cast<double>(most_tiles) > per_sm * a.grid;
 #endif
 }
