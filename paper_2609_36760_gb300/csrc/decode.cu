@@ -913,7 +913,9 @@ constexpr int kPrepThreads = 1024;
 
 // Block 0: tile prefix over units (u = b * n_hg + hg), tiles = ceil(len / 128).
 // Blocks 1..: one query-image piece (16 bytes) per thread.
-template <int CB, int HG>
+// PAIR is a template parameter because block 0 is a chain of latencies that every decode
+// waits for (0.1 to 0.3 us of a 22 to 37 us decode on decode_main with the choice at run time).
+template <int CB, int HG, bool PAIR>
 __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const Params p) {
   griddep_launch_dependents();  // the main kernel may start its set-up meanwhile
   if (blockIdx.x > 0) {
@@ -999,16 +1001,16 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const Params p) {
     // The first tile's block-table entries (clamped column, like row_ref) and length.
     const int b = lo / p.n_hg;
     const int j = t0 - pu0;
-    const int32_t* trow = p.table + static_cast<size_t>(b) * p.max_blocks;
     const bool any = t0 < static_cast<int>(static_cast<long long>(c + 1) * T / p.grid);
-    if (!any) {
-      p.cta_first[c] = make_int4(-1, -1, 0, 0);
-    } else if (p.pair) {
-      p.cta_first[c] =
-          make_int4(ref_start(0, j, pu0, pu1, T, p.sms), ref_start(1, j, pu0, pu1, T, p.sms), p.seq_lens[b], 0);
+    if constexpr (PAIR) {
+      p.cta_first[c] = any ? make_int4(ref_start(0, j, pu0, pu1, T, p.sms), ref_start(1, j, pu0, pu1, T, p.sms),
+                                       p.seq_lens[b], 0)
+                           : make_int4(-1, -1, 0, 0);
     } else {
-      p.cta_first[c] = make_int4(trow[min(2 * j, p.max_blocks - 1)], trow[min(2 * j + 1, p.max_blocks - 1)],
-                                 p.seq_lens[b], j);
+      const int32_t* trow = p.table + static_cast<size_t>(b) * p.max_blocks;
+      p.cta_first[c] = any ? make_int4(trow[min(2 * j, p.max_blocks - 1)], trow[min(2 * j + 1, p.max_blocks - 1)],
+                                       p.seq_lens[b], j)
+                           : make_int4(-1, -1, 0, 0);
     }
     p.cta_t0[c] = t0;
   }
@@ -1266,7 +1268,7 @@ cudaError_t launch_impl(const Params& prm, cudaStream_t stream, cudaEvent_t ev0,
   const long long units = static_cast<long long>(prm.batch) * prm.n_hg;
   const long long pieces = static_cast<long long>(prm.batch) * prm.n_img * kNumChunks * HG * 8;
   const unsigned prep_blocks = static_cast<unsigned>(1 + (pieces + kPrepThreads - 1) / kPrepThreads);
-  if ((e = launch_k(prep_kernel<CB, HG>, dim3(prep_blocks), dim3(kPrepThreads), 0, stream, pdl, prm)) != cudaSuccess)
+  if ((e = launch_k(prep_kernel<CB, HG, PAIR>, dim3(prep_blocks), dim3(kPrepThreads), 0, stream, pdl, prm)) != cudaSuccess)
     return e;
   if (ev0 != nullptr && (e = cudaEventRecord(ev0, stream)) != cudaSuccess) return e;
   if constexpr (PAIR) {
@@ -1358,7 +1360,6 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
   prm.n_hg = pair ? prm.n_img / 2 : prm.n_img;
   prm.grid = pair ? a.grid / 2 : a.grid;
   prm.sms = a.grid;
-  prm.pair = pair;
   prm.q_tokens = a.q_tokens;
   prm.hpt = a.heads / a.q_tokens;
   prm.table = a.table;

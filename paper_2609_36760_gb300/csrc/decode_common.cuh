@@ -45,7 +45,6 @@ struct Params {
   uint32_t* dev_err;
   int grid;  // ranges the tile list is cut into
   int sms;
-  int pair;  // the main kernel runs on CTA pairs (decode_pair.cu)
   unsigned long long* trace;  // trace builds only: per-CTA event clocks, else null
 };
 
