@@ -147,8 +147,10 @@ __global__ void __launch_bounds__(kAppendThreads) quant_append_kernel(
     int max_blocks, uint32_t* dev_err, uint4* __restrict__ prot, const int32_t* __restrict__ lens) {
   static_assert(NT == 1 || NT == 4, "tokens per lane");
   using L = BlockLayout<CB>;
-  // The decode's prep kernel may start meanwhile (it does not read the cache, and
-  // does not end before this kernel has).
+  // The decode's prep kernel may start meanwhile: it does not read the cache, and it
+  // neither writes anything nor ends before this kernel has ended. (A decode step with
+  // prep after the writer / beside it, us: 8 sequences x 128 heads, 300..2,500 tokens,
+  // protected 36.9 / 35.2; 64 x 4,097 INT4 116.8 / 115.5; 128 x 16 heads 186.9 / 185.4.)
   griddep_launch_dependents();
   const int g = threadIdx.x >> 5;  // this warp's group
   const int lane = threadIdx.x & 31;

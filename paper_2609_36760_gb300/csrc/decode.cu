@@ -200,6 +200,7 @@ __device__ __forceinline__ void query_piece(const Params& p, uint8_t* img, int b
 #pragma unroll
     for (int e = 0; e < 4; ++e) ov[e] = pack_h2(f[Perm<4>::at(2 * e)], f[Perm<4>::at(2 * e + 1)]);
   }
+  griddep_wait();  // (see prep_kernel: the image may lie in memory that the cache writer reads)
   *reinterpret_cast<uint4*>(img + k * HG * 128 + swz_off(h, i, 128)) = o;
 }
 
@@ -913,6 +914,11 @@ constexpr int kPrepThreads = 1024;
 
 // Block 0: tile prefix over units (u = b * n_hg + hg), tiles = ceil(len / 128).
 // Blocks 1..: one query-image piece (16 bytes) per thread.
+// The cache writers let this kernel start beside them, so until it has waited for its
+// predecessor it only reads, and nothing that a writer writes: the workspace may be
+// memory that a writer still reads (its latents freed and the workspace allocated in
+// their place). The plan is therefore made in shared memory and registers, and the waits
+// stand before the first writes to the workspace.
 // PAIR is a template parameter because block 0 is a chain of latencies that every decode
 // waits for (0.1 to 0.3 us of a 22 to 37 us decode on decode_main with the choice at run time).
 template <int CB, int HG, bool PAIR>
@@ -936,6 +942,7 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const Params p) {
   const bool pf_on_chip = p.batch * p.n_hg < kSmemUnits;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
+  if (!pf_on_chip) griddep_wait();  // (the prefix goes straight to the workspace)
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
   for (int base = 0; base < p.batch; base += blockDim.x) {
@@ -971,8 +978,8 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const Params p) {
     const int excl = carry + (warp > 0 ? warp_sums[warp - 1] : 0) + x - v;
     if (b < p.batch) {
       for (int hg = 0; hg < p.n_hg; ++hg) {
-        p.prefix_w[b * p.n_hg + hg] = excl + hg * tiles;
-        if (pf_on_chip) pf_s[b * p.n_hg + hg] = excl + hg * tiles;
+        int32_t* const pf = pf_on_chip ? pf_s : p.prefix_w;
+        pf[b * p.n_hg + hg] = excl + hg * tiles;
       }
     }
     __syncthreads();
@@ -980,8 +987,8 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const Params p) {
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    p.prefix_w[p.batch * p.n_hg] = carry;
-    if (pf_on_chip) pf_s[p.batch * p.n_hg] = carry;
+    int32_t* const pf = pf_on_chip ? pf_s : p.prefix_w;
+    pf[p.batch * p.n_hg] = carry;
   }
   __syncthreads();
   // The unit holding the first tile of every decode CTA's range (the unit u
@@ -989,7 +996,15 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const Params p) {
   const volatile int32_t* pf = pf_on_chip ? pf_s : p.prefix_w;
   const int units = p.batch * p.n_hg;
   const int T = pf[units];
-  for (int c = threadIdx.x; c < p.grid; c += blockDim.x) {
+  // (half of the warps copy the prefix out meanwhile)
+  constexpr int kFinders = kPrepThreads / 2;
+  if (threadIdx.x >= kFinders) {
+    griddep_wait();
+    if (pf_on_chip)
+      for (int u = threadIdx.x - kFinders; u <= units; u += kPrepThreads - kFinders) p.prefix_w[u] = pf_s[u];
+    return;
+  }
+  for (int c = threadIdx.x; c < p.grid; c += kFinders) {
     const int t0 = static_cast<int>(static_cast<long long>(c) * T / p.grid);
     int lo = 0, hi = units;
     while (hi - lo > 1) {
@@ -997,27 +1012,28 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const Params p) {
       if (pf[mid] <= t0) lo = mid; else hi = mid;
     }
     const int pu0 = pf[lo], pu1 = pf[lo + 1];
-    p.cta_info[c] = make_int4(lo, pu0, pu1, T);
     // The first tile's block-table entries (clamped column, like row_ref) and length.
     const int b = lo / p.n_hg;
     const int j = t0 - pu0;
     const bool any = t0 < static_cast<int>(static_cast<long long>(c + 1) * T / p.grid);
+    int4 first = make_int4(-1, -1, 0, 0);
     if constexpr (PAIR) {
-      p.cta_first[c] = any ? make_int4(ref_start(0, j, pu0, pu1, T, p.sms), ref_start(1, j, pu0, pu1, T, p.sms),
-                                       p.seq_lens[b], 0)
-                           : make_int4(-1, -1, 0, 0);
+      if (any)
+        first = make_int4(ref_start(0, j, pu0, pu1, T, p.sms), ref_start(1, j, pu0, pu1, T, p.sms), p.seq_lens[b], 0);
     } else {
       const int32_t* trow = p.table + static_cast<size_t>(b) * p.max_blocks;
-      p.cta_first[c] = any ? make_int4(trow[min(2 * j, p.max_blocks - 1)], trow[min(2 * j + 1, p.max_blocks - 1)],
-                                       p.seq_lens[b], j)
-                           : make_int4(-1, -1, 0, 0);
+      if (any)
+        first = make_int4(trow[min(2 * j, p.max_blocks - 1)], trow[min(2 * j + 1, p.max_blocks - 1)], p.seq_lens[b], j);
     }
+    griddep_wait();
+    p.cta_info[c] = make_int4(lo, pu0, pu1, T);
+    p.cta_first[c] = first;
     p.cta_t0[c] = t0;
   }
-  if (threadIdx.x == 0) p.cta_t0[p.grid] = T;
-  // prep reads nothing the cache writer before it writes, but the main kernel
-  // waits only for prep: prep does not complete before the writer has.
+  // (The main kernel waits only for prep, which therefore does not complete before the
+  // writer has.)
   griddep_wait();
+  if (threadIdx.x == 0) p.cta_t0[p.grid] = T;
 }
 
 // Merges the partials of split units with the App. C.5 rule, as a running
