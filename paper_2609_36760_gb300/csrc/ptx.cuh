@@ -374,10 +374,33 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_
 __device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-// Arrives on an mbarrier of another CTA of the cluster, releasing this
-// thread's earlier writes at cluster scope.
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+// Arrival (if pred) on a barrier of any CTA of the cluster, releasing this thread's
+// earlier writes to the threads of its own CTA (the default scope).
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar_cluster_addr, bool pred) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
+      "@q mbarrier.arrive.shared::cluster.b64 _, [%0];\n\t}" ::"r"(bar_cluster_addr),
+      "r"(pred ? 1u : 0u)
+      : "memory");
+}
+// The same releasing them to the whole cluster: the arrival then waits for the thread's
+// outstanding accesses. mbar_test_cluster is its other half, the probe that acquires them.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr, bool pred) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
+      "@q mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n\t}" ::"r"(bar_cluster_addr),
+      "r"(pred ? 1u : 0u)
+      : "memory");
+}
+__device__ __forceinline__ bool mbar_test_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
 }
 // Every thread of both CTAs of the cluster (none may have exited).
 __device__ __forceinline__ void cluster_sync_all() {
@@ -387,31 +410,6 @@ __device__ __forceinline__ void cluster_sync_all() {
 // the cluster that has not exited.
 __device__ __forceinline__ void cluster_arrive_wait() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-// mbar_wait with cluster-scope acquire, for barriers that another CTA of the
-// cluster arrives on after writing into this CTA's shared memory.
-__device__ __forceinline__ int mbar_wait_cluster(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
-                                                 const volatile uint32_t* abort) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  if (ok != 0) return 1;
-  const uint64_t t0 = globaltimer_ns();
-  for (;;) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity), "r"(100000u)
-        : "memory");
-    if (ok != 0) return 1;
-    if (abort != nullptr && *abort != 0u) return -1;
-    if (globaltimer_ns() - t0 > limit_ns) return 0;
-  }
 }
 __device__ __forceinline__ uint4 lds_v4(uint32_t addr) {
   uint4 v;
