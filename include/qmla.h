@@ -185,6 +185,15 @@ size_t qmla_decode_workspace_bytes(int batch, int heads);
  *   workspace_dev   >= qmla_decode_workspace_bytes(batch, heads) bytes, 256-byte aligned;
  *                   contents need no initialisation and are scratch after the call
  * A sequence with seq_lens == 0 gets out = 0 and lse = -inf.
+ *
+ * With 65..128 query rows per sequence (193..256, ...: an even number of 64-row groups)
+ * longer contexts run on pairs of CTAs and shorter ones on single CTAs. The lengths are on
+ * the device, so the choice goes by the longest sequence that block_table has room for,
+ * max_blocks x 64: with a table much wider than its sequences a short decode takes up to
+ * 14% longer than with one cut to what they need (INT2, 16 x 2,000 tokens, 128 heads, a
+ * table for 128K: 43.6 against 38.1 us). Cut the table, or pass max_len to
+ * qmla_mla_decode_ex. Results agree to fp32 rounding (2-norm 2e-5) either way, a raised
+ * softmax reference apart (2^-11).
  */
 int qmla_mla_decode(const void* pool_dev, int c_bits, int num_blocks, const uint16_t* q_latent_dev,
                     const uint16_t* q_pe_dev, int batch, int heads, const int32_t* block_table_dev,
@@ -301,6 +310,10 @@ int qmla_mla_decode_c4r4(const void* pool_dev, int num_blocks, const uint16_t* q
  *                   q_tokens 1..QMLA_MAX_Q_TOKENS query tokens per sequence,
  *                   heads 1..128 per token (as qmla_mla_decode_multi)
  *   prot            sink4/local128 protection buffer or NULL (not with BF16)
+ *   max_len         a bound of seq_lens known on the host, or 0 (max_blocks x 64
+ *                   then). It only chooses between the library's two main kernels
+ *                   (see qmla_mla_decode): a wrong value costs time, never results.
+ *                   (It lies where the structure had padding.)
  *   ev_before_main, ev_after_main
  *                   optional cudaEvent_t (NULL = none): recorded on `stream`
  *                   immediately before and after the main decode kernel of
@@ -324,6 +337,7 @@ typedef struct qmla_decode_desc {
   int heads;
   const int32_t* block_table;
   int max_blocks;
+  int max_len;
   const int32_t* seq_lens;
   const void* prot;
   float softmax_scale;
@@ -406,6 +420,12 @@ int qmla_debug_tile(const void* pool_dev, int cache_kind, int num_blocks, const 
  * 2 s the same way (one site bit per wait, bits 8 and up). */
 #define QMLA_DEVERR_SITE_SOFTMAX (0x100u << 5)
 int qmla_debug_wait_timeout(uint32_t limit_us, uint32_t* dev_err_dev, qmla_stream_t stream);
+
+/* Test hook: the main kernel that qmla_mla_decode_ex runs for this descriptor on a GPU
+ * of `sms` SMs: 0 single CTAs (decode_main), 1 CTA pairs (decode_pair), -1 for a bad
+ * descriptor. Looks at cache_kind, batch, q_tokens, heads, max_blocks, max_len and whether
+ * prot is set; nothing is dereferenced and no device is needed. */
+int qmla_debug_decode_route(const qmla_decode_desc* desc, int sms);
 
 /* Copies the device error word to *host_out after synchronising `stream`. */
 int qmla_read_dev_err(const uint32_t* dev_err_dev, uint32_t* host_out, qmla_stream_t stream);

@@ -33,7 +33,7 @@ class DecodeDesc(ctypes.Structure):
     _fields_ = [("pool", ctypes.c_void_p), ("cache_kind", ctypes.c_int), ("num_blocks", ctypes.c_int),
                 ("q_latent", ctypes.c_void_p), ("q_pe", ctypes.c_void_p), ("batch", ctypes.c_int),
                 ("q_tokens", ctypes.c_int), ("heads", ctypes.c_int), ("block_table", ctypes.c_void_p),
-                ("max_blocks", ctypes.c_int), ("seq_lens", ctypes.c_void_p), ("prot", ctypes.c_void_p),
+                ("max_blocks", ctypes.c_int), ("max_len", ctypes.c_int), ("seq_lens", ctypes.c_void_p), ("prot", ctypes.c_void_p),
                 ("softmax_scale", ctypes.c_float), ("out", ctypes.c_void_p), ("lse", ctypes.c_void_p),
                 ("workspace", ctypes.c_void_p), ("workspace_bytes", ctypes.c_size_t), ("dev_err", ctypes.c_void_p),
                 ("ev_before_main", ctypes.c_void_p), ("ev_after_main", ctypes.c_void_p)]
@@ -92,6 +92,8 @@ def lib():
     L.qmla_mla_decode_multi.restype = i32
     L.qmla_debug_wait_timeout.argtypes = [ctypes.c_uint32, vp, vp]
     L.qmla_debug_wait_timeout.restype = i32
+    L.qmla_debug_decode_route.argtypes = [ctypes.POINTER(DecodeDesc), i32]
+    L.qmla_debug_decode_route.restype = i32
     L.qmla_debug_tile.argtypes = [vp, i32, i32, vp, i32, vp, i32, i32, i32, vp, vp, vp, vp]
     L.qmla_debug_tile.restype = i32
     L.qmla_c4r4_page_bytes.argtypes, L.qmla_c4r4_page_bytes.restype = [], sz
@@ -305,10 +307,12 @@ def static_scratch_bytes() -> int:
 def mla_decode_ex(pool: torch.Tensor, cache_kind, q_latent: torch.Tensor, q_pe: torch.Tensor,
                   block_table: torch.Tensor, seq_lens: torch.Tensor, softmax_scale: float, out: torch.Tensor,
                   lse: torch.Tensor | None, workspace: torch.Tensor, dev_err: torch.Tensor, prot=None,
-                  events: tuple | None = None, stream=None) -> None:
+                  events: tuple | None = None, stream=None, max_len: int = 0) -> None:
     """qmla_mla_decode_ex: cache_kind 4, 2, "c4r4" or "bf16"; q_latent [B,H,512] or
     [B,T,H,512]; events = (before_main, after_main) torch.cuda.Event pair (already
-    recorded once, so that they exist) to record around this call's main kernel."""
+    recorded once, so that they exist) to record around this call's main kernel;
+    max_len = a host-known bound of seq_lens, which chooses the kernel (0: the block
+    table's width does)."""
     if q_latent.dim() == 3:
         B, T, H = q_latent.size(0), 1, q_latent.size(1)
     else:
@@ -319,11 +323,23 @@ def mla_decode_ex(pool: torch.Tensor, cache_kind, q_latent: torch.Tensor, q_pe: 
     d.block_table, d.max_blocks, d.seq_lens = _ptr(block_table), block_table.size(1), _ptr(seq_lens)
     d.prot, d.softmax_scale, d.out, d.lse = _ptr(prot), float(softmax_scale), _ptr(out), _ptr(lse)
     d.workspace, d.workspace_bytes = _ptr(workspace), workspace.nbytes
-    d.dev_err = _ptr(dev_err)
+    d.dev_err, d.max_len = _ptr(dev_err), max_len
     if events is not None:
         d.ev_before_main = ctypes.c_void_p(events[0].cuda_event) if events[0] is not None else None
         d.ev_after_main = ctypes.c_void_p(events[1].cuda_event) if events[1] is not None else None
     _check("qmla_mla_decode_ex", lib().qmla_mla_decode_ex(ctypes.byref(d), _stream(stream)))
+
+
+def debug_decode_route(cache_kind, batch: int, heads: int, max_blocks: int, q_tokens: int = 1, protect: bool = False,
+                       max_len: int = 0, sms: int = 152) -> str:
+    """qmla_debug_decode_route: the main kernel of such a decode on a GPU of `sms` SMs."""
+    d = DecodeDesc()
+    d.cache_kind, d.batch, d.q_tokens, d.heads = CACHE_KINDS[cache_kind], batch, q_tokens, heads
+    d.max_blocks, d.max_len, d.prot = max_blocks, max_len, 16 if protect else None
+    r = lib().qmla_debug_decode_route(ctypes.byref(d), sms)
+    if r < 0:
+        raise ValueError("bad decode description")
+    return ("decode_main", "decode_pair")[r]
 
 
 def read_dev_err(dev_err: torch.Tensor, stream=None) -> int:

@@ -83,7 +83,7 @@ int decode_common(const void* pool, int kind, int num_blocks, const uint16_t* q_
                   int batch, int heads, const int32_t* table, int max_blocks, const int32_t* seq_lens,
                   float softmax_scale, float* out, float* lse, void* workspace, size_t workspace_bytes,
                   uint32_t* dev_err, qmla_stream_t stream, const void* prot = nullptr, int q_tokens = 1,
-                  void* ev_before_main = nullptr, void* ev_after_main = nullptr) {
+                  void* ev_before_main = nullptr, void* ev_after_main = nullptr, int max_len = 0) {
   int st = decode_checks(pool, num_blocks, q_latent, q_pe, batch, heads, table, max_blocks, seq_lens, softmax_scale,
                          out, lse, workspace, prot, q_tokens);
   if (st != QMLA_OK) return st;
@@ -102,6 +102,7 @@ int decode_common(const void* pool, int kind, int num_blocks, const uint16_t* q_
   a.heads = heads;
   a.table = table;
   a.max_blocks = max_blocks;
+  a.max_len = max_len;
   a.seq_lens = seq_lens;
   a.softmax_scale = softmax_scale;
   a.out = out;
@@ -324,6 +325,19 @@ int qmla_debug_tile(const void* pool_dev, int cache_kind, int num_blocks, const 
   return e == cudaSuccess ? QMLA_OK : cuda_fail(e);
 }
 
+int qmla_debug_decode_route(const qmla_decode_desc* d, int sms) {
+  if (desc_checks(d) != QMLA_OK || d->batch < 1 || d->max_blocks < 1 || sms < 1) return -1;
+  qmla::DecodeArgs a;
+  a.cache_kind = d->cache_kind;
+  a.batch = d->batch;
+  a.heads = d->q_tokens * d->heads;
+  a.max_blocks = d->max_blocks;
+  a.max_len = d->max_len;
+  a.prot = d->prot;
+  a.grid = sms;
+  return qmla::decode_on_pairs(a) ? 1 : 0;
+}
+
 int qmla_debug_wait_timeout(uint32_t limit_us, uint32_t* dev_err_dev, qmla_stream_t stream) {
   if (dev_err_dev == nullptr || limit_us < 1u || limit_us > 1000000u) return QMLA_ERR_INVALID_ARG;
   DevInfo di;
@@ -348,7 +362,7 @@ int qmla_mla_decode_ex(const qmla_decode_desc* d, qmla_stream_t stream) {
   return decode_common(d->pool, d->cache_kind, d->num_blocks, d->q_latent, d->q_pe, d->batch, d->q_tokens * d->heads,
                        d->block_table, d->max_blocks, d->seq_lens, d->softmax_scale, d->out, d->lse, d->workspace,
                        d->workspace_bytes, d->dev_err, stream, d->prot, d->q_tokens, d->ev_before_main,
-                       d->ev_after_main);
+                       d->ev_after_main, d->max_len);
 }
 
 int qmla_last_cuda_error(void) { return g_last_cuda_error; }

@@ -31,7 +31,7 @@
 //                  At a segment end the softmax warps write the final output, or
 //                  an unnormalised partial (m, l, o) when the unit is split.
 //                  (decode_pair takes its place for even numbers of 64-head groups
-//                  over longer contexts, see use_pair.)
+//                  over longer contexts, see decode_on_pairs.)
 //   combine_kernel merges the partials of split units with
 //                  m = max m_j, l = sum e^(m_j - m) l_j, O = sum e^(m_j - m) o_j / l
 //                  (combine_wide_kernel for a few long units).
@@ -1312,35 +1312,47 @@ cudaError_t launch_hg(int hg, bool pair, const Params& prm, cudaStream_t stream,
   return launch_impl<CB, 64, PROT, false>(prm, stream, ev0, ev1);
 }
 
-// Whether a decode runs on CTA pairs (decode_pair.cu): two 64-head groups per unit, and
-// enough tiles per SM, by the most that the block table allows, to pay for the pair's
-// fixed part (the reference tiles above all). The pair gains most where decode_main's
-// workers have most to do per row: measured on one GB300 (decode alone, 128 heads,
-// decode_main against the pair, us; in brackets the tiles per SM):
+}  // namespace
+
+#ifdef QMLA_TRACE_BUILD
+unsigned long long* g_trace_buf = nullptr;  // set by set_trace_buffer
+#endif
+
+// Two 64-row groups per unit, and enough tiles per SM to pay for the pair's fixed part
+// (the reference tiles above all). The lengths are on the device, so the tiles are counted
+// by the caller's bound of them (max_len) or else by the block table's width: the most
+// that the call can have. The pair gains most where decode_main's workers have most to do
+// per row: measured on one GB300 (decode alone, 128 heads, decode_main against the pair,
+// us; in brackets the tiles per SM of a table just wide enough):
 //   INT4             16 x 4,000 (7) 51.9 / 53.0   32 x 4,000 (13) 72.6 /  70.4
 //   INT2            32 x 4,000 (13) 72.8 / 76.9   64 x 4,097 (28) 124.3 / 122.6
 //   the paper's page 16 x 4,000 (7) 57.3 / 58.3   64 x 2,000 (13)  86.0 /  82.8
 //   INT4, protected  4 x 4,000 (1.7) 30.9 / 26.1  32 x 4,000 (13)  87.9 /  78.5
 //   page, protected  4 x 4,000 (1.7) 31.5 / 26.5  32 x 4,000 (13)  96.3 /  84.9
 //   BF16 cache       4 x 4,000 (1.7) 32.7 / 27.4  32 x 4,000 (13) 128.4 /  95.0
-bool use_pair(const DecodeArgs& a) {
+// What a table of 2,048 columns (128K tokens) costs shorter sequences without max_len,
+// since it sends them to the pair (the same two times; protected and BF16 rows lose 5%
+// at most, nearly all of them gain):
+//               1 x 1,000    16 x 1,000   16 x 2,000   64 x 256     64 x 1,000   64 x 2,000
+//   INT4        18.9 / 19.4  34.5 / 36.5  38.6 / 41.9  31.5 / 33.8  51.8 / 54.1  75.1 / 73.9
+//   INT2        19.0 / 19.8  34.1 / 37.5  38.1 / 43.6  31.1 / 34.8  51.5 / 57.0  75.4 / 79.4
+//   the page    20.2 / 19.8  35.8 / 38.0  41.2 / 44.8  33.4 / 35.3  57.9 / 59.0  85.6 / 82.5
+// (A choice on the device, both kernels launched and one leaving at once, cost 1.4 to 4
+// us in every call, whichever was chosen.)
+bool decode_on_pairs(const DecodeArgs& a) {
 #ifdef QMLA_TRACE_BUILD
   return false;  // the timeline is decode_main's
 #else
   const int groups = (a.heads + 63) / 64;
   if (groups % 2 != 0 || a.grid < 2) return false;
-  const long long most_tiles = static_cast<long long>(a.batch) * groups * ((static_cast<long long>(a.max_blocks) + 1) / 2);
+  const long long width = (static_cast<long long>(a.max_blocks) + 1) / 2;
+  const long long tiles = a.max_len > 0 ? (static_cast<long long>(a.max_len) + kTileTokens - 1) / kTileTokens : width;
+  const long long most_tiles = static_cast<long long>(a.batch) * groups * (tiles < width ? tiles : width);
   const bool heavy_rows = a.cache_kind == 16 || a.prot != nullptr;
   const double per_sm = heavy_rows ? 1.5 : (a.cache_kind == kC4R4 ? 10.0 : a.cache_kind == 4 ? 12.0 : 18.0);
   return static_cast<double>(most_tiles) > per_sm * a.grid;
 #endif
 }
-
-}  // namespace
-
-#ifdef QMLA_TRACE_BUILD
-unsigned long long* g_trace_buf = nullptr;  // set by set_trace_buffer
-#endif
 
 int head_group_size(int heads) { return heads <= 16 ? 16 : (heads <= 32 ? 32 : 64); }
 
@@ -1371,7 +1383,7 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
   prm.q_pe = reinterpret_cast<const __nv_bfloat16*>(a.q_pe);
   prm.batch = a.batch;
   prm.heads = a.heads;
-  const bool pair = use_pair(a);
+  const bool pair = decode_on_pairs(a);
   prm.n_img = (a.heads + hg - 1) / hg;
   prm.n_hg = pair ? prm.n_img / 2 : prm.n_img;
   prm.grid = pair ? a.grid / 2 : a.grid;

@@ -39,6 +39,7 @@ struct DecodeArgs {
   int q_tokens = 1;  // query tokens per sequence (the last q_tokens positions, causal among them)
   const int32_t* table;
   int max_blocks;
+  int max_len = 0;  // the caller's bound of the lengths, or 0
   const int32_t* seq_lens;
   float softmax_scale;
   float* out;
@@ -51,6 +52,8 @@ struct DecodeArgs {
   cudaEvent_t ev_after_main = nullptr;
 };
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream);
+// Whether this decode runs on CTA pairs (decode_pair.cu) or on decode_main.
+bool decode_on_pairs(const DecodeArgs& a);
 // Test hook: tile j of sequence b as the decode kernel builds it, [128][576] fp16.
 cudaError_t launch_tile_dump(const DecodeArgs& a, int b, int j, uint16_t* out, cudaStream_t stream);
 // Test hook: a decode wait that runs out after limit_ns (see qmla_debug_wait_timeout).
