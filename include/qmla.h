@@ -32,6 +32,15 @@
  *   32-bit error word `dev_err_dev` (QMLA_DEVERR_*). The offending access is
  *   skipped; no call traps or aborts. Read the word with qmla_read_dev_err.
  * - bf16 / fp16 tensors are passed as uint16_t bit patterns.
+ * - Plain launches on one stream keep stream order, whatever memory they share. Kernels
+ *   that a caller launches with programmatic stream serialisation have to know two things.
+ *   The cache writers let their dependents start at once (griddepcontrol
+ *   .launch_dependents), so such a kernel right behind a writer runs beside it: it must
+ *   execute griddepcontrol.wait, even if it uses nothing of the cache, for a decode
+ *   behind it waits for that kernel alone. And a decode's first kernel is such a launch
+ *   itself: it reads q_latent, q_pe, block_table and seq_lens before it waits, so a kernel
+ *   right before the decode must not let its dependents start before it has written
+ *   those. (Everything else a decode reads, and all that it writes, comes after the wait.)
  *
  * Cache format (this library's own 64-token block, little-endian)
  * ----------------------------------------------------------------
