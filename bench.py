@@ -40,6 +40,8 @@ METRIC = "low-bit MLA decode KV-tokens/s and µs/step on 1 GB300; % of roofline"
 UNIT = "KV-tokens/s"
 DEFAULT_WORKLOAD = "dsv3_b64_h128_l4096_int4"
 TAU = 1.0 / math.sqrt(192.0)
+KERNELS = {"decode_main": "decode_main: one CTA per SM (qmla_mla_decode)",
+           "decode_pair": "decode_pair: one CTA pair per two SMs (qmla_mla_decode)"}
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}
 
 
@@ -61,7 +63,7 @@ def parse(argv=None):
     ap.add_argument("--no-configs", action="store_true",
                     help="skip the other workloads (configs) measured after the headline one")
     ap.add_argument("--trace", default=None, metavar="NPZ",
-                    help="instead of timing: build the trace library, trace one decode step's main kernel, print "
+                    help="instead of timing: build the trace library, trace one decode step on decode_main, print "
                          "the per-tile stage breakdown and save the raw clock64 stamps to NPZ")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
@@ -160,37 +162,37 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def profile_traffic(kernel_file_hash: str, workload: str, bf16: bool = False, protect: bool = False,
+def profile_traffic(kernel_file_hash: str, kernel: str, workload: str, bf16: bool = False, protect: bool = False,
                     c4r4: bool = False, q_tokens: int = 1):
     """The committed ncu record of DRAM bytes per main-kernel launch for this
-    workload and cache variant, if it was taken on the current kernel sources;
-    otherwise None."""
-    p = os.path.join(ROOT, "profiles", "decode_main_traffic.json")
+    kernel (decode_main or decode_pair), workload and cache variant, if it was
+    taken on the current kernel sources; otherwise None."""
+    p = os.path.join(ROOT, "profiles", "decode_traffic.json")
     if not os.path.exists(p):
         return None
     with open(p) as f:
         d = json.load(f)
-    if d.get("decode_cu_sha256") != kernel_file_hash:
+    if d.get("decode_sources_sha256") != kernel_file_hash:
         return None
     for r in d.get("records", []):
-        if (r.get("workload") == workload and bool(r.get("bf16_cache")) == bool(bf16)
+        if (r.get("kernel") == kernel and r.get("workload") == workload and bool(r.get("bf16_cache")) == bool(bf16)
                 and bool(r.get("protect")) == bool(protect) and bool(r.get("c4r4")) == bool(c4r4)
                 and int(r.get("q_tokens", 1)) == q_tokens):
             return r
     return None
 
 
-# The sources decode_main is compiled from (its translation unit and headers).
-DECODE_MAIN_SOURCES = ("common.cuh", "decode.cu", "decode_common.cuh", "decode_pair.cu", "kernels.h", "ptx.cuh")
+# The sources the main decode kernels are compiled from (translation units and headers).
+DECODE_SOURCES = ("common.cuh", "decode.cu", "decode_common.cuh", "decode_pair.cu", "kernels.h", "ptx.cuh")
 
 
-def decode_cu_hash() -> str:
-    """sha256 over the sources decode_main is compiled from (and the public
-    header they include), so a traffic figure taken on another version of the
-    kernel is not used."""
+def decode_sources_hash() -> str:
+    """sha256 over the sources the main decode kernels are compiled from (and the
+    public header they include), so a traffic figure taken on another version of
+    a kernel is not used."""
     d = os.path.join(ROOT, "paper_2609_36760_gb300", "csrc")
     h = hashlib.sha256()
-    paths = [os.path.join(d, n) for n in DECODE_MAIN_SOURCES] + [os.path.join(ROOT, "include", "qmla.h")]
+    paths = [os.path.join(d, n) for n in DECODE_SOURCES] + [os.path.join(ROOT, "include", "qmla.h")]
     for path in paths:
         with open(path, "rb") as f:
             h.update(os.path.basename(path).encode() + b"\0" + f.read())
@@ -288,6 +290,11 @@ class Workspace:
 
     def cache_kind(self):
         return "bf16" if self.bf16 else ("c4r4" if self.c4r4 else self.w.c_bits)
+
+    def kernel(self) -> str:
+        """The main kernel that this workload's decode runs on this GPU."""
+        return self.Q.debug_decode_route(self.cache_kind(), self.w.batch, self.w.heads, self.table.shape[1],
+                                         q_tokens=self.q_tokens, protect=self.protect, sms=self.Q.num_sms())
 
     def decode(self, d: dict, out, lse, events=None):
         """One decode call through the variant's own entry point; with events
@@ -431,12 +438,12 @@ def run_native(args, ws_world: int, rank: int, local: int):
     value = whole_job_value(ws_world, tok_per_step, ms_step_max)
 
     roof = roofline(w, t["lens0"], args.bf16_cache, state.c4r4, args.q_tokens, ms_main)
-    prof = profile_traffic(decode_cu_hash(), args.workload, args.bf16_cache, args.protect, state.c4r4,
-                           args.q_tokens)
+    prof = profile_traffic(decode_sources_hash(), state.kernel(), args.workload, args.bf16_cache, args.protect,
+                           state.c4r4, args.q_tokens)
     roof["traffic"] = prof["dram_bytes_per_launch"] if prof else None
     if prof:
-        roof["traffic_source"] = "profiles/decode_main_traffic.json: " + prof["source"]
-    roof["kernel"] = "decode_main"
+        roof["traffic_source"] = "profiles/decode_traffic.json: " + prof["source"]
+    roof["kernel"] = state.kernel()
 
     # end to end through the public API with host buffers
     e2e = None
@@ -449,7 +456,7 @@ def run_native(args, ws_world: int, rank: int, local: int):
         "dtype": "f16", "data": "synthetic (seeded generators, workloads/synthetic.py)",
         "config": {"workload": w.name, "batch_per_gpu": w.batch, "heads": w.heads, "c_bits": w.c_bits,
                    "pe_bits": 4, "cache": cache_name(w, args.bf16_cache, args.protect, state.c4r4),
-                   "q_tokens_per_seq": args.q_tokens, "kernel": "one CTA per SM (qmla_mla_decode)",
+                   "q_tokens_per_seq": args.q_tokens, "kernel": KERNELS[state.kernel()],
                    "kv_tokens_per_step_per_gpu": tok_per_step, "l2": "flushed (256 MB write) before every timed step",
                    "parallelism": f"replicas x{ws_world} (independent sequences)"},
         "us_per_step": round(ms_step_max * 1e3, 2),
@@ -506,7 +513,8 @@ def run_configs(dev, flush, K: int) -> dict:
         ms_step = sum(step_ms) / len(step_ms)
         ms_main = sum(main_ms) / len(main_ms)
         roof = roofline(state.w, t["lens0"], bf16, False, 1, ms_main)
-        prof = profile_traffic(decode_cu_hash(), name, bf16)
+        roof["kernel"] = state.kernel()
+        prof = profile_traffic(decode_sources_hash(), roof["kernel"], name, bf16)
         roof["traffic"] = prof["dram_bytes_per_launch"] if prof else None
         qs = statistics.quantiles(step_ms, n=10) if len(step_ms) >= 10 else [min(step_ms)] * 9
         r = {"cache": cache_name(w, bf16, False, False), "batch": w.batch, "heads": w.heads,
@@ -515,7 +523,7 @@ def run_configs(dev, flush, K: int) -> dict:
                                   "p10": round(qs[0] * 1e3, 2), "p90": round(qs[-1] * 1e3, 2)},
              "kv_tokens_per_s": round(t["tokens_per_step"] / (ms_step * 1e-3), 1),
              "kv_tokens_per_step": t["tokens_per_step"], "step_parts_us": t["parts_us"],
-             "roofline": {k: roof[k] for k in ("bound", "achieved", "peak", "unit", "frac", "kernel_us",
+             "roofline": {k: roof[k] for k in ("kernel", "bound", "achieved", "peak", "unit", "frac", "kernel_us",
                                               "roofline_us", "algorithmic_bytes", "algorithmic_flops", "traffic")},
              "hbm_gbs_of_step": round(roof["algorithmic_bytes"] / (ms_step * 1e-3) / 1e9, 1),
              "gpu_launches": state.launches_per_step() * Kc,
@@ -775,11 +783,11 @@ def main_trace_summary(ev):
 
 
 def run_trace(args):
-    """Per-tile event timeline of the main decode kernel from the trace build
-    (-DQMLA_TRACE_BUILD: clock64 stamps at pipeline events of the first eight
-    CTAs, written through the buffer given to qmla_trace_set). Stamps are per-SM
-    clocks: only differences within one CTA mean anything (event numbers in
-    main_trace_summary)."""
+    """Per-tile event timeline of decode_main, on which the trace build runs every
+    decode, also those that decode_pair takes otherwise (-DQMLA_TRACE_BUILD:
+    clock64 stamps at pipeline events of the first eight CTAs, written through the
+    buffer given to qmla_trace_set). Stamps are per-SM clocks: only differences
+    within one CTA mean anything (event numbers in main_trace_summary)."""
     import ctypes
 
     import numpy as np

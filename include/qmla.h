@@ -40,7 +40,8 @@
  *   behind it waits for that kernel alone. And a decode's first kernel is such a launch
  *   itself: it reads q_latent, q_pe, block_table and seq_lens before it waits, so a kernel
  *   right before the decode must not let its dependents start before it has written
- *   those. (Everything else a decode reads, and all that it writes, comes after the wait.)
+ *   those. (Everything else a decode reads, and all that it writes but bits of the
+ *   error word, comes after the wait.)
  *
  * Cache format (this library's own 64-token block, little-endian)
  * ----------------------------------------------------------------
