@@ -46,28 +46,6 @@ __device__ __forceinline__ uint32_t quant_code(float x, float s, float z, float 
   return static_cast<uint32_t>(fminf(fmaxf(rintf(__fdiv_rn(x, s) + z), 0.0f), m));
 }
 
-// Two fp32 operations per instruction.
-__device__ __forceinline__ uint64_t f32x2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // The codes clip(rne(x / s + z), 0, m) of eight bf16 values (four words of two),
 // as four words with one code in each half, without a division per value: y =
 // RN(1 / s), q = RN(x y) corrected once by its exact residual x - q s (P.
@@ -136,9 +114,9 @@ constexpr int kAppendThreads = kGroups * 32;
 // destination up and works out its scale, and shuffles hand them round. Groups
 // outside codes8's argument (quotients above 2^14, infinite values or scales) and
 // the fp32 RoPE scale of the paper's page, whose codes are defined by the rounded
-// fp32 quotient, divide value by value. 32,797 tokens (INT4) take 16.6 us, 2.9 TB/s of
-// 6.8; a warp per (token, group) with two coordinates per lane and a division per
-// code took 61.5.
+// fp32 quotient, divide value by value. 32,797 tokens of eight ragged prompts (INT4, calls
+// on buffers larger together than L2) take 16.5 us, 2.9 TB/s of 6.8; a warp per (token,
+// group) with two coordinates per lane and a division per code took 61.5.
 template <int CB, int NT, bool VEC>
 __global__ void __launch_bounds__(kAppendThreads) quant_append_kernel(
     uint8_t* __restrict__ pool, int num_blocks, const uint32_t* __restrict__ latent,
@@ -337,9 +315,10 @@ void launch_quant(void* pool, int num_blocks, const uint16_t* latent, const uint
 }
 
 // Tokens from which a lane takes four: below, one token per lane spreads the
-// tokens over more SMs and ends sooner. One GB300, INT4 / the paper's page, four
-// against one: 4,096 tokens 3.6 against 3.6 / 4.4 against 3.8 us, 8,192 5.0 against
-// 5.8 / 5.8 against 6.2, 32,768 13.8 against 18.5 / 16.8 against 19.6.
+// tokens over more SMs and ends sooner. One GB300, INT4 / the paper's page, eight
+// prompts of equal length, buffers larger together than L2, four against one: 4,096
+// tokens 4.1 against 3.9 / 5.4 against 4.5 us, 8,192 5.8 against 6.3 / 7.1 against 7.1,
+// 32,768 15.1 against 19.5 / 19.8 against 20.7.
 constexpr int kFourPerLane = 8192;
 
 template <int CB>

@@ -268,25 +268,7 @@ __device__ void pair_dequant(const Params& p, PairSched sc, uint32_t smem, PairC
 }
 
 // ------------------------------------------------------------------- softmax
-// Two fp32 operations per instruction.
-__device__ __forceinline__ uint64_t pair2(uint32_t a, uint32_t b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
-  return r;
-}
-__device__ __forceinline__ float lo2(uint64_t a) { return __uint_as_float(static_cast<uint32_t>(a)); }
-__device__ __forceinline__ float hi2(uint64_t a) { return __uint_as_float(static_cast<uint32_t>(a >> 32)); }
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-// acc + w.lo + w.hi with w a pair of fp16 values.
+// lo += w.lo, hi += w.hi with w a pair of fp16 values.
 __device__ __forceinline__ void add_h2(float& lo, float& hi, uint32_t w) {
   asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tadd.rn.f32.f16 %0, l, %0;\n\tadd.rn.f32.f16 %1, h, %1;\n\t}"
       : "+f"(lo), "+f"(hi)
@@ -301,7 +283,9 @@ __device__ __forceinline__ void load_scores(uint32_t t_s, uint64_t (&x)[16]) {
   tmem_ld32(t_s + 32, b);
   tmem_ld_wait();
 #pragma unroll
-  for (int i = 0; i < 16; ++i) x[i] = add2(pair2(a[2 * i], a[2 * i + 1]), pair2(b[2 * i], b[2 * i + 1]));
+  for (int i = 0; i < 16; ++i)
+    x[i] = add2(f32x2(__uint_as_float(a[2 * i]), __uint_as_float(a[2 * i + 1])),
+                f32x2(__uint_as_float(b[2 * i]), __uint_as_float(b[2 * i + 1])));
 }
 // Largest scaled score among the row's first `vis` of 32 columns (-inf if none).
 __device__ __forceinline__ float scores_max(const uint64_t (&x)[16], float sl2, int vis) {
@@ -416,8 +400,8 @@ __device__ void pair_softmax(const Params& p, PairSched sc, uint32_t smem, PairC
   int vis = 0;
   bool full = true;
   auto weights = [&]() {  // whether a weight is above 2^8 (as rounded)
-    const uint64_t ss = pair2(__float_as_uint(sl2), __float_as_uint(sl2));
-    const uint64_t nm = pair2(__float_as_uint(-m), __float_as_uint(-m));
+    const uint64_t ss = f32x2(sl2, sl2);
+    const uint64_t nm = f32x2(-m, -m);
     __half2 top = __float2half2_rn(0.0f);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -597,6 +581,9 @@ __device__ void pair_softmax(const Params& p, PairSched sc, uint32_t smem, PairC
     // Through the P tiles (free until the next tile's weights), 32 columns at a time, so
     // that a warp stores whole 128-byte lines: a row per lane would touch 32 lines with
     // every store, 8k cycles a segment instead of about 2k.
+    // (A warp's piece of them lies under other warps' weights. Those of the next segment
+    // do not come before every warp is done: a segment that follows another starts its
+    // unit, so its first tile renews the reference, with an exchange of all four warps.)
     const int h0 = (sc.g * 2 + rank) * static_cast<int>(kRows) + (warp & 1) * 32;  // the warp's first row
     const size_t orow0 = whole ? static_cast<size_t>(sc.b) * p.heads + h0
                                : (static_cast<size_t>(pair) + sc.unit) * 128 + rank * kRows + (warp & 1) * 32;
@@ -850,46 +837,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1) dec
   griddep_wait();
 
   // (Each role makes its own schedule: one made before the branch, held across the
-  // register split, spilled 244 instead of 60 bytes; 64 x 4,097 tokens, INT4: 120.8 us
+  // register split, spilled 244 bytes instead of 76 at most; 64 x 4,097 tokens, INT4: 120.8 us
   // instead of 115.1, BF16 168.5 instead of 163.3, INT2 32 x 32,768 386 instead of 368.)
-  // (Each role makes its own schedule: one made before the branch and held across the
-  // register split spilled up to 244 bytes; the INT4 step then took 120.8 us.)
   if (warp < kSoftWarps) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftRegs));
     PairSched sc;
     sc.init(p, pair);
     pair_softmax<CB>(p, sc, smem, ctl, tmem, rank, warp, lane, pair);
   } else {
-   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
-   if (warp < kMmaWarp) {
-    PairSched sc;
-    sc.init(p, pair);
-    pair_dequant<CB, PROT>(p, sc, smem, ctl, rank, warp - kSoftWarps, lane);
-   } else if (warp > kPrefetchWarp) {
-    asm volatile("exit;");
-   } else if (elect_one()) {  // the issuers are single threads
-    PairSched sc;
-    sc.init(p, pair);
-    if (warp == kMmaWarp) {
-      if (rank == 0) {
-        pair_mma(p, sc, sm, smem, ctl, tmem);
-      } else {
-        pair_query(p, sc, sm, ctl, rank);
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kOtherRegs));
+    if (warp < kMmaWarp) {
+      PairSched sc;
+      sc.init(p, pair);
+      pair_dequant<CB, PROT>(p, sc, smem, ctl, rank, warp - kSoftWarps, lane);
+    } else if (warp > kPrefetchWarp) {
+      asm volatile("exit;");
+    } else if (elect_one()) {  // the issuers are single threads
+      PairSched sc;
+      sc.init(p, pair);
+      if (warp == kMmaWarp) {
+        if (rank == 0) {
+          pair_mma(p, sc, sm, smem, ctl, tmem);
+        } else {
+          pair_query(p, sc, sm, ctl, rank);
+        }
+      } else if (rank != 0) {
+        pair_prefetch<CB>(p, sc, ctl);
       }
-    } else if (rank != 0) {
-      pair_prefetch<CB>(p, sc, ctl);
+      if (warp == kMmaWarp && rank == 0) {
+        // Every MMA must have landed before TMEM and shared memory are released;
+        // this wait ignores the abort flag.
+        umma2_commit_local(&ctl.fin);
+        wait_ok(mbar_wait(&ctl.fin, 0, kWaitNs, nullptr), kSiteMmaFin, ctl, p.dev_err);
+      }
+    } else {
+      // The other lanes leave: parked at a re-convergence point they delay the wake-up of
+      // the elected one from its waits by more than a thousand cycles.
+      asm volatile("exit;");
     }
-    if (warp == kMmaWarp && rank == 0) {
-      // Every MMA must have landed before TMEM and shared memory are released;
-      // this wait ignores the abort flag.
-      umma2_commit_local(&ctl.fin);
-      wait_ok(mbar_wait(&ctl.fin, 0, kWaitNs, nullptr), kSiteMmaFin, ctl, p.dev_err);
-    }
-   } else {
-    // The other lanes leave: parked at a re-convergence point they delay the wake-up of
-    // the elected one from its waits by more than a thousand cycles.
-    asm volatile("exit;");
-   }
   }
   griddep_launch_dependents();  // the merge may be scheduled as CTAs finish
   tc_fence_before();
