@@ -12,14 +12,15 @@
 // and its scores are double-buffered, and separate warps dequantise, do the
 // softmax and issue the MMAs, so that the tiles' phases overlap.
 //
-// decode_main is bound by the shared-memory port: per 128 tokens and 64 rows its MMAs
-// read 3,390 and its workers write 1,280 wavefronts of 128 bytes, and the softmax leaves
-// the port idle. Here the MMAs read 2,500 and the warps write about 1,200 per 128 tokens
-// and 64 rows of each CTA, beside the softmax. What bounds the kernel now is the softmax
-// warps' turn, about 3.1k cycles per 64-token tile, most of it waits on shared memory and
-// TMEM behind the other warps' bursts. One GB300, a decode step of 64 sequences x 128
-// heads x 4,097 tokens, decode_main / this: INT4 129.0 / 115.1 us, the paper's page with
-// protection 174.2 / 138.1, BF16 237.4 / 163.3; INT2, 32 x 32,768 tokens: 395.5 / 368.2.
+// Per 128 tokens and 64 rows decode_main's MMAs read 3,390 and its workers write 1,370
+// wavefronts of 128 bytes of shared memory, one phase after the other; here the MMAs read
+// 2,590 and the warps write 1,430, the reference tiles' among them, beside the softmax
+// (ncu, the INT4 step below). Of 3.35k cycles per 64-token tile the tensor pipe then is
+// active in 33% and the shared-memory port busy in 65%; the rest is the softmax warps'
+// turn, mostly waits on shared memory and TMEM behind the other warps' bursts. One GB300, a
+// decode step of 64 sequences x 128 heads x 4,097 tokens, decode_main / this: INT4 129.0 /
+// 116.5 us, the paper's page with protection 174.2 / 136.8, BF16 237.4 / 165.1; INT2, 32 x
+// 32,768 tokens: 395.5 / 363.
 // (A second softmax group, one per alternate tile, was slower: 152 us on the INT4 step,
 // its warps' extra waits and registers cost more than their overlap gave.)
 //
